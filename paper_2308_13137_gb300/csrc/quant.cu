@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256, 4) lwc_fwd_kernel(LwcFwdArgs a) {
       gb = __shfl_sync(0xffffffffu, gb, 0);
     }
     const QState qs = omq_qstate(M, m, ga, gb, Q, a.eps);
-    int iM = 0x7fffffff, im = 0x7fffffff;        // first index of the max / min held by this lane
+    int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;        // first index of the max / min held by this lane
     for (int it0 = 0; it0 < iters; it0 += 4) {
       uint4 raw[4];
 #pragma unroll
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(256, 4) lwc_fwd_kernel(LwcFwdArgs a) {
       im = min(im, __shfl_xor_sync(0xffffffffu, im, off));
     }
     if (lane == 0) {
-      a.h[o] = qs.h; a.z[o] = (int32_t)qs.z; a.imax[o] = iM; a.imin[o] = im;
+      a.h[o] = qs.h; a.z[o] = (int32_t)qs.z; a.imax[o] = omq_saved_index(iM, 0); a.imin[o] = omq_saved_index(im, 0);
       if (a.ga_out) { a.ga_out[o] = ga; a.gb_out[o] = gb; }
       if (a.M_out) { a.M_out[o] = M; a.m_out[o] = m; }
     }
@@ -226,7 +226,9 @@ __global__ void __launch_bounds__(256, 4) lwc_fwd_kernel(LwcFwdArgs a) {
           const QState qs = omq_qstate(r.M, r.m, ga, gb, Q, a.eps);
           if (lane == leader) {
             const int64_t k = o * ngroups + gi;
-            a.h[k] = qs.h; a.z[k] = (int32_t)qs.z; a.imax[k] = r.iM; a.imin[k] = r.im;
+            const int g0 = (int)(gi * gsz);
+            a.h[k] = qs.h; a.z[k] = (int32_t)qs.z;
+            a.imax[k] = omq_saved_index(r.iM, g0); a.imin[k] = omq_saved_index(r.im, g0);
             if (a.ga_out) { a.ga_out[k] = ga; a.gb_out[k] = gb; }
             if (a.M_out) { a.M_out[k] = r.M; a.m_out[k] = r.m; }
           }
@@ -327,7 +329,7 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
       }
     }
     // first column of the max and of the min: this lane's, then the group's
-    int iM = 0x7fffffff, im = 0x7fffffff;
+    int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
     if constexpr (SCALED) {
 #pragma unroll
       for (int i = 31; i >= 0; --i) {
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
         const uint32_t lo = mask & 0xffffu, hi = mask >> 16;
         const int i0 = lo ? 2 * (__ffs(lo) - 1) : 64, i1 = hi ? 2 * (__ffs(hi) - 1) + 1 : 64;
         const int i = min(i0, i1);
-        return i < 64 ? (int)col0 + (i >> 3) * LPG * 8 + (i & 7) : 0x7fffffff;
+        return i < 64 ? (int)col0 + (i >> 3) * LPG * 8 + (i & 7) : OMQ_NO_INDEX;
       };
       iM = first(eM);
       im = first(em);
@@ -361,7 +363,10 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
     }
     const QState qs = omq_qstate(M, m, ga, gb, Q, a.eps);
     if (valid) {
-      if (sub == 0) { a.h[k] = qs.h; a.z[k] = (int32_t)qs.z; a.imax[k] = iM; a.imin[k] = im; }
+      if (sub == 0) {                            // col0 is the group's first column here
+        a.h[k] = qs.h; a.z[k] = (int32_t)qs.z;
+        a.imax[k] = omq_saved_index(iM, (int)col0); a.imin[k] = omq_saved_index(im, (int)col0);
+      }
       if (sub == LPG - 1) {
         if (a.ga_out) { a.ga_out[k] = ga; a.gb_out[k] = gb; }
         if (a.M_out) { a.M_out[k] = M; a.m_out[k] = m; }
@@ -433,7 +438,7 @@ __global__ void __launch_bounds__(NT, !SCALED ? 1024 / NT : NT == 128 ? (CPT > 6
   float logit = 0.f;                                 // warp 0: even lanes gamma's, odd ones beta's
   if (warp == 0) {
     if (a.lwc) logit = (lane & 1) ? a.bl[o] : a.gl[o];
-    if (lane < 2) sidx[lane] = 0x7fffffff;
+    if (lane < 2) sidx[lane] = OMQ_NO_INDEX;
   }
   float wt[SCALED ? CPT : 1][8];
   float M = -INFINITY, m = INFINITY, dot = 0.f;
@@ -516,7 +521,7 @@ __global__ void __launch_bounds__(NT, !SCALED ? 1024 / NT : NT == 128 ? (CPT > 6
   bM = state[3]; bm = state[4];
   const bool small = state[5] != 0.f;
   if (M == bM || m == bm) {
-    int iM = 0x7fffffff, im = 0x7fffffff;
+    int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
 #pragma unroll
     for (int j = CPT - 1; j >= 0; --j) {
       const int c = j * NT + tid;
@@ -534,8 +539,8 @@ __global__ void __launch_bounds__(NT, !SCALED ? 1024 / NT : NT == 128 ? (CPT > 6
         if (v[e] == bm) im = c * 8 + e;
       }
     }
-    if (iM != 0x7fffffff) atomicMin(&sidx[0], iM);
-    if (im != 0x7fffffff) atomicMin(&sidx[1], im);
+    if (iM != OMQ_NO_INDEX) atomicMin(&sidx[0], iM);
+    if (im != OMQ_NO_INDEX) atomicMin(&sidx[1], im);
   }
 #pragma unroll
   for (int j = 0; j < CPT; ++j) {
@@ -552,7 +557,7 @@ __global__ void __launch_bounds__(NT, !SCALED ? 1024 / NT : NT == 128 ? (CPT > 6
     else lwc_store_at<false>(a, o * nchunk + c, v, qs, Q);
   }
   __syncthreads();
-  if (tid == 0) { a.imax[o] = sidx[0]; a.imin[o] = sidx[1]; }
+  if (tid == 0) { a.imax[o] = omq_saved_index(sidx[0], 0); a.imin[o] = omq_saved_index(sidx[1], 0); }
 }
 
 template <int NT, bool SCALED>

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(NT, MINB) act_fwd_rows(ActFwdArgs a) {
   const int64_t t = blockIdx.x;
   const bool quant = a.abits < 16;
   const float Q = (float)((1 << (quant ? a.abits : 1)) - 1);
-  if (tid == 0) { sidx[0] = 0x7fffffff; sidx[1] = 0x7fffffff; }
+  if (tid == 0) { sidx[0] = OMQ_NO_INDEX; sidx[1] = OMQ_NO_INDEX; }
   float4 raw[VPT];
 #pragma unroll
   for (int j = 0; j < VPT; ++j) {                   // every load of the row first
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(NT, MINB) act_fwd_rows(ActFwdArgs a) {
 #pragma unroll
     for (int w = 1; w < NW; ++w) { M = fmaxf(M, red[0][w]); m = fminf(m, red[1][w]); }
     if (lM == M || lm == m) {
-      int iM = 0x7fffffff, im = 0x7fffffff;
+      int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
 #pragma unroll
       for (int k = NE - 1; k >= 0; --k) {
         const int64_t vi = (int64_t)(k >> 2) * NT + tid;
@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(NT, MINB) act_fwd_rows(ActFwdArgs a) {
           if (val[k >> 2][k & 3] == m) im = (int)(4 * vi) + (k & 3);
         }
       }
-      if (iM != 0x7fffffff) atomicMin(&sidx[0], iM);
-      if (im != 0x7fffffff) atomicMin(&sidx[1], im);
+      if (iM != OMQ_NO_INDEX) atomicMin(&sidx[0], iM);
+      if (im != OMQ_NO_INDEX) atomicMin(&sidx[1], im);
     }
     qs = omq_qstate(M, m, 1.f, 1.f, Q, a.eps);
     small = omq_small_quot(qs);
@@ -171,7 +171,8 @@ __global__ void __launch_bounds__(NT, MINB) act_fwd_rows(ActFwdArgs a) {
   if (!quant) return;
   __syncthreads();                                  // first indices final
   if (tid == 0) {
-    a.h[t] = qs.h; a.z[t] = (int32_t)qs.z; a.imax[t] = sidx[0]; a.imin[t] = sidx[1];
+    a.h[t] = qs.h; a.z[t] = (int32_t)qs.z;
+    a.imax[t] = omq_saved_index(sidx[0], 0); a.imin[t] = omq_saved_index(sidx[1], 0);
   }
 }
 
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__(NT) act_fwd_smem(ActFwdArgs a) {
   const float Q = (float)((1 << (quant ? a.abits : 1)) - 1);
   const float* xr = a.X + t * a.ldx;
   const float* ur = P == AP_SWIGLU ? a.U + t * a.ldu : nullptr;
-  if (tid == 0) { sidx[0] = 0x7fffffff; sidx[1] = 0x7fffffff; }
+  if (tid == 0) { sidx[0] = OMQ_NO_INDEX; sidx[1] = OMQ_NO_INDEX; }
   QState qs{};
   float lM = -INFINITY, lm = INFINITY;
   for (int i0 = tid; i0 < nv; i0 += 4 * NT) {
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(NT) act_fwd_smem(ActFwdArgs a) {
   }
   qs = omq_qstate(M, m, 1.f, 1.f, Q, a.eps);
   const bool small = omq_small_quot(qs);
-  int iM = 0x7fffffff, im = 0x7fffffff;
+  int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
   const bool holder = lM == M || lm == m;
   for (int vi = tid; vi < nv; vi += NT) {
     const float4 r = row4[vi];
@@ -259,10 +260,13 @@ __global__ void __launch_bounds__(NT) act_fwd_smem(ActFwdArgs a) {
     }
     act_store4(a, t, vi, v, qs, Q, true, small);
   }
-  if (iM != 0x7fffffff) atomicMin(&sidx[0], iM);
-  if (im != 0x7fffffff) atomicMin(&sidx[1], im);
+  if (iM != OMQ_NO_INDEX) atomicMin(&sidx[0], iM);
+  if (im != OMQ_NO_INDEX) atomicMin(&sidx[1], im);
   __syncthreads();
-  if (tid == 0) { a.h[t] = qs.h; a.z[t] = (int32_t)qs.z; a.imax[t] = sidx[0]; a.imin[t] = sidx[1]; }
+  if (tid == 0) {
+    a.h[t] = qs.h; a.z[t] = (int32_t)qs.z;
+    a.imax[t] = omq_saved_index(sidx[0], 0); a.imin[t] = omq_saved_index(sidx[1], 0);
+  }
 }
 
 // ================================================================================================
@@ -872,7 +876,7 @@ __global__ void __launch_bounds__(NT) qkv_fwd_rows(QkvArgs a) {
   const float* sa = seg == 0 ? a.sa_exp : a.sa;
   const bool let = seg < 2 && a.sa_exp != nullptr;
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (tid == 0) { sidx[0] = 0x7fffffff; sidx[1] = 0x7fffffff; }
+  if (tid == 0) { sidx[0] = OMQ_NO_INDEX; sidx[1] = OMQ_NO_INDEX; }
   float4 ca = z4, cb = z4, x1[PPT], x2[PPT];
   if (seg < 2) {                                       // (cos, sin) of the four frequencies
     const float* cs = a.cs + (int64_t)t * 128 + 8 * (tid & 15);
@@ -928,7 +932,7 @@ __global__ void __launch_bounds__(NT) qkv_fwd_rows(QkvArgs a) {
 #pragma unroll
     for (int w = 1; w < NW; ++w) { M = fmaxf(M, red[0][w]); m = fminf(m, red[1][w]); }
     if (lM == M || lm == m) {                          // only the holders of an extreme search its first index
-      int iM = 0x7fffffff, im = 0x7fffffff;
+      int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
 #pragma unroll
       for (int j = 0; j < PPT; ++j) {
         const int p = j * NT + tid;
@@ -941,8 +945,8 @@ __global__ void __launch_bounds__(NT) qkv_fwd_rows(QkvArgs a) {
           if (v2[j][e] == m) im = min(im, pair_elem(p) + 64 + e);
         }
       }
-      if (iM != 0x7fffffff) atomicMin(&sidx[0], iM);
-      if (im != 0x7fffffff) atomicMin(&sidx[1], im);
+      if (iM != OMQ_NO_INDEX) atomicMin(&sidx[0], iM);
+      if (im != OMQ_NO_INDEX) atomicMin(&sidx[1], im);
     }
     qs = omq_qstate(M, m, 1.f, 1.f, Q, a.eps);
     small = omq_small_quot(qs);
@@ -964,7 +968,8 @@ __global__ void __launch_bounds__(NT) qkv_fwd_rows(QkvArgs a) {
   __syncthreads();                                     // first indices final
   if (tid == 0) {
     const int64_t k = (int64_t)seg * a.T + t;
-    a.h[k] = qs.h; a.z[k] = (int32_t)qs.z; a.imax[k] = sidx[0]; a.imin[k] = sidx[1];
+    a.h[k] = qs.h; a.z[k] = (int32_t)qs.z;
+    a.imax[k] = omq_saved_index(sidx[0], 0); a.imin[k] = omq_saved_index(sidx[1], 0);
   }
 }
 
