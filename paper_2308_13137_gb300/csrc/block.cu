@@ -588,6 +588,12 @@ omq_status block_bwd(Ctx& c, const float* x, const float* y, const float* y_fp, 
   return OMQ_OK;
 }
 
+// the kernels read these in float4s: s1, d1, s2, d2, and so, do where no copy is expanded to the query heads
+bool let_aligned(const omq_block_params& p, bool expanded) {
+  return omq_aligned16(p.s1) && omq_aligned16(p.d1) && omq_aligned16(p.s2) && omq_aligned16(p.d2) &&
+         (expanded || (omq_aligned16(p.so) && omq_aligned16(p.do_)));
+}
+
 omq_status make_ctx(Ctx& c, omq_stream_t stream, const omq_block_shape* shape, const omq_block_weights* w,
                     const omq_block_params* theta, void* workspace, size_t ws_bytes, const omq_qcfg* cfg, bool bwd) {
   OMQ_TRY(check_block(shape, cfg));
@@ -598,9 +604,11 @@ omq_status make_ctx(Ctx& c, omq_stream_t stream, const omq_block_shape* shape, c
     OMQ_REQUIRE(theta->gamma_qkv && theta->beta_qkv && theta->gamma_o && theta->beta_o && theta->gamma_gu &&
                     theta->beta_gu && theta->gamma_d && theta->beta_d,
                 OMQ_ERR_INVALID_ARG);
-  if (cfg->let)
+  if (cfg->let) {
     OMQ_REQUIRE(theta->s1 && theta->d1 && theta->so && theta->do_ && theta->sa && theta->s2 && theta->d2,
                 OMQ_ERR_INVALID_ARG);
+    OMQ_REQUIRE(let_aligned(*theta, shape->n_heads > shape->n_kv) && omq_aligned16(theta->sa), OMQ_ERR_ALIGN);
+  }
   Carve dry{nullptr, 0};
   BlockWS tmp;
   carve_block(dry, *shape, *cfg, tmp, bwd);
@@ -702,6 +710,10 @@ omq_status omq_qlinear_fwd(omq_stream_t stream, int64_t T, int64_t Cin, int64_t 
   OMQ_REQUIRE(X && W && Y && sv && sv->w_hat && sv->x_hat && sv->b_tilde, OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(!cfg->let || (s && delta), OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(Cin % 8 == 0 && Cout % 8 == 0, OMQ_ERR_ALIGN);
+  OMQ_REQUIRE(omq_aligned16(X) && omq_aligned16(W) && omq_aligned16(Y) && omq_aligned16(sv->w_hat) &&
+                  omq_aligned16(sv->x_hat) && (!(B || cfg->let) || omq_aligned16(sv->b_tilde)) &&
+                  (!cfg->let || (omq_aligned16(s) && omq_aligned16(delta))),
+              OMQ_ERR_ALIGN);
   cudaStream_t st = (cudaStream_t)stream;
   const int g = cfg->group == 0 ? (int)Cin : cfg->group;
   OMQ_REQUIRE(Cin % g == 0, OMQ_ERR_SHAPE);
@@ -784,7 +796,10 @@ omq_status omq_qlinear_bwd(omq_stream_t stream, int64_t T, int64_t Cin, int64_t 
   const bool let = cfg->let != 0;
   OMQ_REQUIRE(!let || (s && delta && ds && ddelta), OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(workspace && ws_bytes >= omq_qlinear_workspace_size(T, Cin, Cout, cfg), OMQ_ERR_WORKSPACE);
-  OMQ_REQUIRE(omq_aligned16(workspace) && omq_aligned16(dY), OMQ_ERR_ALIGN);
+  OMQ_REQUIRE(omq_aligned16(workspace) && omq_aligned16(dY) && omq_aligned16(X) && omq_aligned16(W) &&
+                  omq_aligned16(dX) && omq_aligned16(sv->x_hat) &&
+                  (!(dX || let) || omq_aligned16(sv->w_hat)) && (!let || (omq_aligned16(s) && omq_aligned16(delta))),
+              OMQ_ERR_ALIGN);
   cudaStream_t st = (cudaStream_t)stream;
   const int group = cfg->group == 0 ? (int)Cin : cfg->group;
   OMQ_REQUIRE(Cin % 8 == 0 && Cout % 8 == 0, OMQ_ERR_ALIGN);
@@ -834,6 +849,7 @@ extern "C" omq_status omq_let_stats_accumulate(omq_stream_t stream, const omq_bl
   OMQ_REQUIRE(x && stats && stats->a_absmax && stats->a_sum && stats->q_absmax && stats->k_absmax &&
                   stats->o_absmax && stats->o_sum && stats->b_absmax && stats->b_sum,
               OMQ_ERR_INVALID_ARG);
+  OMQ_REQUIRE(omq_aligned16(x), OMQ_ERR_ALIGN);
   omq_qcfg fp{};
   fp.wbits = 16; fp.abits = 16; fp.group = 0; fp.let = 0; fp.h_eps = 1e-5f; fp.accumulate = 0;
   fp.dev_status = dev_status;
@@ -936,6 +952,9 @@ extern "C" omq_status omq_block_fold_pack(omq_stream_t stream, const omq_block_s
                     out->b_qkv && out->b_o && out->b_gu && out->ln1_gain && out->ln1_bias && out->ln2_gain &&
                     out->ln2_bias && out->sa,
                 OMQ_ERR_INVALID_ARG);
+  OMQ_REQUIRE(omq_aligned16(w->wqkv) && omq_aligned16(w->wo) && omq_aligned16(w->wgu) && omq_aligned16(w->wd) &&
+                  (!let || let_aligned(*theta, true)),
+              OMQ_ERR_ALIGN);
   OMQ_REQUIRE(workspace && ws_bytes >= omq_block_pack_workspace_size(shape, cfg) && omq_aligned16(workspace),
               OMQ_ERR_WORKSPACE);
   cudaStream_t st = (cudaStream_t)stream;

@@ -1607,6 +1607,7 @@ omq_status omq_lwc_fakequant_fwd(omq_stream_t stream, int64_t Cout, int64_t Cin,
   OMQ_REQUIRE(W, OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(Cin % 8 == 0 && omq_aligned16(W) && (!Wq || omq_aligned16(Wq)), OMQ_ERR_ALIGN);
   OMQ_REQUIRE(!codes || ((uintptr_t)codes & 7) == 0, OMQ_ERR_ALIGN);
+  OMQ_REQUIRE(omq_aligned16(s) && (!Bt || omq_aligned16(bias_delta)), OMQ_ERR_ALIGN);
   const int g = cfg->group == 0 ? (int)Cin : cfg->group;
   OMQ_REQUIRE(Cin % g == 0, OMQ_ERR_SHAPE);
   if (cfg->wbits < 16) OMQ_REQUIRE(h && z && argmax && argmin && gamma_logit && beta_logit, OMQ_ERR_INVALID_ARG);
@@ -1656,6 +1657,7 @@ omq_status omq_act_quant_per_token(omq_stream_t stream, int64_t T, int64_t C, co
   OMQ_REQUIRE(T > 0 && C > 0, OMQ_ERR_SHAPE);
   OMQ_REQUIRE(X && Xq, OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(C % 8 == 0 && omq_aligned16(X) && omq_aligned16(Xq), OMQ_ERR_ALIGN);
+  OMQ_REQUIRE(omq_aligned16(s) && omq_aligned16(delta) && ((uintptr_t)codes & 3) == 0, OMQ_ERR_ALIGN);
   if (cfg->abits < 16) OMQ_REQUIRE(h && z && argmax && argmin, OMQ_ERR_INVALID_ARG);
   ActFwdArgs a{};
   a.producer = (s || delta) ? AP_LET : AP_PLAIN;
@@ -1677,12 +1679,16 @@ omq_status omq_act_quant_per_token_bwd(omq_stream_t stream, int64_t T, int64_t C
   OMQ_REQUIRE(T > 0 && C > 0, OMQ_ERR_SHAPE);
   OMQ_REQUIRE(X && dXq, OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE(C % 8 == 0 && omq_aligned16(X) && omq_aligned16(dXq), OMQ_ERR_ALIGN);
+  OMQ_REQUIRE(omq_aligned16(s) && omq_aligned16(delta) && omq_aligned16(dX), OMQ_ERR_ALIGN);
   if (cfg->abits < 16) OMQ_REQUIRE(h && z && argmax && argmin, OMQ_ERR_INVALID_ARG);
   OMQ_REQUIRE((!ds && !ddelta) || (s && delta), OMQ_ERR_INVALID_ARG);
   const bool need_ws = ds || ddelta;
   const int rows = need_ws ? act_bwd_rows(T, C, 4, 64) : 4;
   const int64_t P = (T + rows - 1) / rows;           // partial rows, at most the workspace's (T + 3) / 4
-  if (need_ws) OMQ_REQUIRE(workspace && ws_bytes >= omq_act_bwd_workspace_size(T, C), OMQ_ERR_WORKSPACE);
+  if (need_ws) {
+    OMQ_REQUIRE(workspace && ws_bytes >= omq_act_bwd_workspace_size(T, C), OMQ_ERR_WORKSPACE);
+    OMQ_REQUIRE(omq_aligned16(workspace), OMQ_ERR_ALIGN);
+  }
   cudaStream_t st = (cudaStream_t)stream;
   ActBwdArgs a{};
   a.producer = (s || delta) ? AP_LET : AP_PLAIN;

@@ -110,3 +110,50 @@ def test_block_workspace_sizes():
     ws8 = _lib.omq_block_workspace_size(s, _cfg(wbits=4, abits=4, group=0, let=1, pbits=8))
     assert ws < ws8 < ws + 16 * sh.n_heads * sh.T * 4
     assert _lib.omq_block_workspace_size(s, _cfg(wbits=4, abits=4, group=0, let=1, pbits=12)) == 0
+
+
+def _refused(fn, args, at, off, code=3):
+    """fn with args is refused with `code` when the pointer at position `at` is moved by `off` bytes."""
+    a = list(args)
+    a[at] = FAKE + off
+    return fn(*a) == code
+
+
+def test_vector_pointers_must_be_aligned():
+    """Pointers that the kernels read or write in 16-byte vectors are refused on the host when they are not 16-byte
+    aligned."""
+    L = _lib.lib()
+    c = ctypes.byref(_cfg(abits=4, group=0, let=1))
+    act_f = [None, 4, 512, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, c]
+    for i in (3, 4, 5, 6):                                   # X, s, delta, Xq
+        assert _refused(L.omq_act_quant_per_token, act_f, i, 4)
+    assert _refused(L.omq_act_quant_per_token, act_f, 7, 2)  # codes, written four at a time
+    act_b = [None, 4, 512, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, 1 << 30, c]
+    for i in (3, 4, 5, 10, 11, 14):                          # X, s, delta, dXq, dX, workspace
+        assert _refused(L.omq_act_quant_per_token_bwd, act_b, i, 8)
+    lwc_f = [None, 64, 512, FAKE, FAKE, None, FAKE, FAKE, FAKE, None, FAKE, FAKE, FAKE, FAKE, FAKE, None, FAKE, c]
+    for i in (3, 4, 8, 14):                                  # W, s, Wq, bias_delta
+        assert _refused(L.omq_lwc_fakequant_fwd, lwc_f, i, 8)
+    sv = _lib.omq_qlinear_saved(*[FAKE] * 11)
+    ql_f = [None, 4, 512, 64, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, ctypes.byref(sv), c]
+    for i in (4, 5, 7, 8, 11):                               # X, W, s, delta, Y
+        assert _refused(L.omq_qlinear_fwd, ql_f, i, 8)
+    ql_b = [None, 4, 512, 64, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, ctypes.byref(sv), FAKE, FAKE, FAKE, FAKE, FAKE, FAKE, FAKE,
+            1 << 30, c]
+    for i in (4, 5, 6, 7, 11, 12, 17):                       # X, W, s, delta, dY, dX, workspace
+        assert _refused(L.omq_qlinear_bwd, ql_b, i, 8)
+
+
+def test_let_vectors_must_be_aligned():
+    """The block's LET vectors: all of them with a kv head per query head; with shared kv heads so and do are
+    expanded to copies first, so theirs does not matter."""
+    L, c = _lib.lib(), ctypes.byref(_cfg(abits=4, group=0, let=1))
+    w = _lib.omq_block_weights(FAKE, FAKE, FAKE, FAKE)
+    for n_kv, names in ((2, ["s1", "d1", "so", "do_", "sa", "s2", "d2"]), (1, ["s1", "d1", "sa", "s2", "d2"])):
+        s = _lib.omq_block_shape(16, 256, 2, n_kv, 128, 384, 1e-6, 1e4)
+        for n in names + [None]:
+            th = _lib.omq_block_params(*[FAKE] * len(_lib.PARAM_FIELDS))
+            if n:
+                setattr(th, n, FAKE + 8)
+            e = L.omq_block_forward(None, ctypes.byref(s), ctypes.byref(w), ctypes.byref(th), FAKE, FAKE, FAKE, 0, c)
+            assert e == (3 if n else 7), (n_kv, n, e)        # OMQ_ERR_ALIGN, or the workspace of no bytes
