@@ -719,12 +719,12 @@ template <int P, int NT>
 static omq_status act_fwd_smem_go(cudaStream_t st, const ActFwdArgs& a) {
   auto kern = act_fwd_smem<P, NT>;
   const size_t smem = a.abits < 16 ? (size_t)a.C * 4 : 0;
-  static size_t smem_set = 40 * 1024;                 // with its static part a CTA has 48 KB without asking
-  if (smem > smem_set) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return OMQ_ERR_CUDA;
-    smem_set = smem;
-  }
+  // With its static part a CTA has 48 KB without asking.  What is asked for is the longest row's, on every call: the
+  // limit belongs to the current device, and one that followed the rows seen so far could be lowered by another
+  // host thread between a call and its launch
+  if (smem > 40 * 1024 &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 32 * 1024) != cudaSuccess)
+    return OMQ_ERR_CUDA;
   kern<<<(unsigned)a.T, NT, smem, st>>>(a);
   OMQ_LAUNCH_CHECK();
   return OMQ_OK;
