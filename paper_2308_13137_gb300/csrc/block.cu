@@ -778,6 +778,7 @@ QlinearWS carve_qlinear(Carve& c, int64_t T, int64_t Cin, int64_t Cout, const om
 }  // namespace
 
 size_t omq_qlinear_workspace_size(int64_t T, int64_t Cin, int64_t Cout, const omq_qcfg* cfg) {
+  if (T <= 0 || Cin <= 0 || Cout <= 0) return 0;
   Carve c{nullptr, 0};
   omq_qcfg any{};                               // without a configuration: enough for every one of them
   any.group = 8;

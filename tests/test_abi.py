@@ -157,3 +157,19 @@ def test_let_vectors_must_be_aligned():
                 setattr(th, n, FAKE + 8)
             e = L.omq_block_forward(None, ctypes.byref(s), ctypes.byref(w), ctypes.byref(th), FAKE, FAKE, FAKE, 0, c)
             assert e == (3 if n else 7), (n_kv, n, e)        # OMQ_ERR_ALIGN, or the workspace of no bytes
+
+
+def test_qlinear_workspace_of_bad_shapes():
+    """A shape without tokens or columns has no workspace, whatever the group (a query in a process of its own: it
+    used to end the process)."""
+    import subprocess
+    import sys
+    code = ("import ctypes, sys; sys.path.insert(0, %r); from paper_2308_13137_gb300 import _lib; L = _lib.lib()\n"
+            "for g in (0, 128):\n"
+            "    c = _lib.make_cfg(4, 16, g, 0)\n"
+            "    for s in ((4, 0, 64), (4, 512, 0), (0, 512, 64), (-1, 512, 64), (4, -512, 64)):\n"
+            "        for p in (ctypes.byref(c), None):\n"
+            "            assert L.omq_qlinear_workspace_size(*s, p) == 0, (s, g)\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code % root], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stderr)
