@@ -220,6 +220,8 @@ omq_status omq_qlinear_bwd(omq_stream_t stream, int64_t T, int64_t Cin, int64_t 
                            const omq_qlinear_saved* saved, const float* dY, float* dX,
                            float* dgamma, float* dbeta, float* ds, float* ddelta,
                            void* workspace, size_t ws_bytes, const omq_qcfg* cfg);
+/* Depends on the shape alone: the buffer serves every configuration (cfg may be NULL).  0 for a
+ * non-positive size. */
 size_t omq_qlinear_workspace_size(int64_t T, int64_t Cin, int64_t Cout, const omq_qcfg* cfg);
 /* Element counts of the omq_qlinear_saved arrays, in the struct's field order (w_hat, h_w, z_w,
  * imax_w, imin_w, x_hat, h_a, z_a, imax_a, imin_a, b_tilde), written to sizes[0..10] (host array

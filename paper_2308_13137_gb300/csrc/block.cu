@@ -25,12 +25,17 @@ typedef __nv_bfloat16 bf16;
 
 struct QState4 { float* h; int32_t* z; int32_t* imax; int32_t* imin; float* ga; float* gb; float* M; float* m; };
 
-// Scratch (floats) of the fused weight-gradient + LWC backward of one [Cout, Cin] weight over T tokens
-int64_t lwc_fused_scratch_elems(int64_t T, int64_t Cout, int64_t Cin, int64_t group) {
-  const int64_t bn = gemm_lwc_tile(Cout, Cin, T, group).bn;
-  const int64_t ntn = bn ? 2 * ((Cin + bn - 1) / bn) : 0;                      // row partials per row
+// Scratch (floats) of the fused weight-gradient + LWC backward of one [Cout, Cin] weight with ntn row partials a row
+int64_t lwc_fused_elems(int64_t Cout, int64_t Cin, int64_t ntn) {
   return 2 * ((Cout + 31) / 32) * Cin + 3 * Cout * ntn + 4 * Cout + 64;
 }
+// over T tokens
+int64_t lwc_fused_scratch_elems(int64_t T, int64_t Cout, int64_t Cin, int64_t group) {
+  const int64_t bn = gemm_lwc_tile(Cout, Cin, T, group).bn;
+  return lwc_fused_elems(Cout, Cin, bn ? 2 * ((Cin + bn - 1) / bn) : 0);
+}
+// the same for the configuration that needs most: the narrowest tile, 64 columns, has the most row partials
+int64_t lwc_fused_scratch_max(int64_t Cout, int64_t Cin) { return lwc_fused_elems(Cout, Cin, 2 * ((Cin + 63) / 64)); }
 
 bool lwc_fused_ok(int64_t T, int64_t Cout, int64_t Cin, int group, bool let_terms) {
   return (group == Cin || !let_terms) && gemm_lwc_tile(Cout, Cin, T, group).bn > 0;
@@ -754,23 +759,20 @@ omq_status omq_qlinear_saved_sizes(int64_t T, int64_t Cin, int64_t Cout, const o
 namespace {
 struct QlinearWS {
   bf16* dYb;                   // dY in bf16
-  float* dWh;                  // dW_hat, only where the LWC backward does not run in the product's epilogue
+  float* dWh;                  // dW_hat; where the LWC backward runs in the product's epilogue, the groups' states
   float* dXh;
   float* dB;                   // gradient of the LET bias
-  float *ga, *gb, *M, *m;      // per group
   float* part;
 };
-QlinearWS carve_qlinear(Carve& c, int64_t T, int64_t Cin, int64_t Cout, const omq_qcfg& cfg) {
-  const int group = cfg.group == 0 ? (int)Cin : cfg.group;
-  const int64_t ng = Cout * (Cin / group);
+// one layout for every configuration: a buffer of the queried size serves any group and LET setting
+QlinearWS carve_qlinear(Carve& c, int64_t T, int64_t Cin, int64_t Cout) {
   QlinearWS w;
   w.dYb = c.take<bf16>(T * Cout);
-  w.dWh = lwc_fused_ok(T, Cout, Cin, group, cfg.let != 0) ? nullptr : c.take<float>(Cout * Cin);
+  w.dWh = c.take<float>(Cout * Cin);
   w.dXh = c.take<float>(T * Cin);
   w.dB = c.take<float>(Cout);
-  w.ga = c.take<float>(ng); w.gb = c.take<float>(ng); w.M = c.take<float>(ng); w.m = c.take<float>(ng);
   int64_t pe = imax64((int64_t)lwc_bwd_scratch_bytes(Cout, Cin) / 4 + 64, 2 * ((T + 3) / 4) * Cin);
-  pe = imax64(pe, lwc_fused_scratch_elems(T, Cout, Cin, group));
+  pe = imax64(pe, lwc_fused_scratch_max(Cout, Cin));
   pe = imax64(pe, colsum_rows_parts(T) * Cout);
   w.part = c.take<float>(pe);
   return w;
@@ -779,10 +781,9 @@ QlinearWS carve_qlinear(Carve& c, int64_t T, int64_t Cin, int64_t Cout, const om
 
 size_t omq_qlinear_workspace_size(int64_t T, int64_t Cin, int64_t Cout, const omq_qcfg* cfg) {
   if (T <= 0 || Cin <= 0 || Cout <= 0) return 0;
+  (void)cfg;
   Carve c{nullptr, 0};
-  omq_qcfg any{};                               // without a configuration: enough for every one of them
-  any.group = 8;
-  carve_qlinear(c, T, Cin, Cout, cfg && cfg->group >= 0 ? *cfg : any);
+  carve_qlinear(c, T, Cin, Cout);
   return c.off + 256;
 }
 
@@ -806,16 +807,20 @@ omq_status omq_qlinear_bwd(omq_stream_t stream, int64_t T, int64_t Cin, int64_t 
   OMQ_REQUIRE(Cin % 8 == 0 && Cout % 8 == 0, OMQ_ERR_ALIGN);
   OMQ_REQUIRE(Cin % group == 0, OMQ_ERR_SHAPE);
   Carve c{(uint8_t*)workspace, 0};
-  const QlinearWS w = carve_qlinear(c, T, Cin, Cout, *cfg);
+  const QlinearWS w = carve_qlinear(c, T, Cin, Cout);
   OMQ_TRY(to_bf16_launch(st, dY, T, Cout, w.dYb, w.part, let ? w.dB : nullptr));
   // the strengths and extremes of the groups, which the saved state does not hold, then dW_hat = dY^T X_hat
   // with the LWC backward in its epilogue: storing dW_hat and walking it again took 121 us more of the
-  // 752 us of a 2048 x 4096 -> 11008 linear
-  LwcBwdArgs la{};
-  la.W = (const bf16*)W; la.Cout = Cout; la.Cin = Cin; la.group = group; la.s = let ? s : nullptr;
-  la.gl = gamma_logit; la.bl = beta_logit; la.imax = sv->imax_w; la.imin = sv->imin_w;
-  OMQ_TRY(lwc_state_launch(st, la, w.ga, w.gb, w.M, w.m));
-  const QState4 qw{sv->h_w, sv->z_w, sv->imax_w, sv->imin_w, w.ga, w.gb, w.M, w.m};
+  // 752 us of a 2048 x 4096 -> 11008 linear.  Where it is stored all the same, that pass forms them itself.
+  QState4 qw{sv->h_w, sv->z_w, sv->imax_w, sv->imin_w, nullptr, nullptr, nullptr, nullptr};
+  if (lwc_fused_ok(T, Cout, Cin, group, let)) {
+    const int64_t ng = Cout * (Cin / group);    // four arrays in dW_hat's room, groups of at least 8 columns
+    qw.ga = w.dWh; qw.gb = w.dWh + ng; qw.M = w.dWh + 2 * ng; qw.m = w.dWh + 3 * ng;
+    LwcBwdArgs la{};
+    la.W = (const bf16*)W; la.Cout = Cout; la.Cin = Cin; la.group = group; la.s = let ? s : nullptr;
+    la.gl = gamma_logit; la.bl = beta_logit; la.imax = sv->imax_w; la.imin = sv->imin_w;
+    OMQ_TRY(lwc_state_launch(st, la, qw.ga, qw.gb, qw.M, qw.m));
+  }
   OMQ_TRY(lwc_bwd_dw(st, T, w.dYb, (const bf16*)sv->x_hat, (const bf16*)W, Cout, Cin, *cfg, let ? s : nullptr, nullptr,
                      gamma_logit, beta_logit, qw, dgamma, dbeta, nullptr, let ? w.dB : nullptr, let ? ds : nullptr,
                      let ? ddelta : nullptr, cfg->accumulate, w.part, w.dWh, cfg->dev_status));

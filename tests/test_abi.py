@@ -173,3 +173,13 @@ def test_qlinear_workspace_of_bad_shapes():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", code % root], capture_output=True, text=True)
     assert r.returncode == 0, (r.returncode, r.stderr)
+
+
+def test_qlinear_workspace_serves_every_configuration():
+    """One size per shape, whatever the group and the LET setting: a buffer sized once is accepted with any of them."""
+    L = _lib.lib()
+    for T, Cin, Cout in ((256, 512, 512), (1, 8, 8), (300, 520, 136), (2048, 4096, 11008)):
+        sizes = {L.omq_qlinear_workspace_size(T, Cin, Cout, ctypes.byref(_cfg(group=g, let=let)))
+                 for g in (0, 8, 32, 64, 128, 256) for let in (0, 1)}
+        sizes.add(L.omq_qlinear_workspace_size(T, Cin, Cout, None))
+        assert len(sizes) == 1 and sizes.pop() > 2 * T * Cout + 4 * Cout * Cin + 4 * T * Cin
