@@ -303,7 +303,7 @@ template <int P>
 __device__ __forceinline__ float act_xt(const ActBwdArgs& a, float x, float u, float dl, float sv, float rstd) {
   float v;
   if (P == AP_SWIGLU) v = silu(x) * u;
-  else if (P == AP_RMS_LET) v = x * rstd;
+  else if (P == AP_RMS_LET) v = __fmul_rn(x, rstd);   // rounded before delta is taken off, as in the forward
   else v = x;
   if (P == AP_LET || P == AP_RMS_LET) {
     if (a.delta) v = v - dl;
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(NT, MINB) act_bwd_stream(ActBwdArgs a) {
               sg[e] = __frcp_rn(1.f + expf(-x));
               v[e] = (x * sg[e]) * f4get(u4[jj], e);
             } else {
-              v[e] = P == AP_RMS_LET ? x * rstd : x;
+              v[e] = P == AP_RMS_LET ? __fmul_rn(x, rstd) : x;
             }
           }
           if (LETP) {
@@ -854,9 +854,10 @@ omq_status act_bwd_launch(cudaStream_t st, const ActBwdArgs& a0) {
 // of 16, so all of them turn by the same four angles.
 // ================================================================================================
 __device__ __forceinline__ int pair_elem(int p) { return (p >> 4) * 128 + 4 * (p & 15); }   // its first element
+// the rounding is spelled out, so that the backward re-forms the forward's values bit for bit
 __device__ __forceinline__ void rope_pair(float a1, float a2, float c, float s, float& r1, float& r2) {
-  r1 = a1 * c - a2 * s;
-  r2 = a2 * c + a1 * s;
+  r1 = fmaf(a1, c, -__fmul_rn(a2, s));
+  r2 = fmaf(a2, c, __fmul_rn(a1, s));
 }
 
 // One CTA per (token, q | k | v), the segment in registers: bound by the row's own latency (loads, two
