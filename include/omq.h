@@ -120,7 +120,7 @@ size_t omq_lwc_bwd_workspace_size(int64_t Cout, int64_t Cin);
  * per-token MinMax quantizer (Eq. 2 with gamma = beta = 1, one group per row, N = cfg->abits).
  *   X [T, C] fp32 -> Xq [T, C] bf16 = (q - z) h (or bf16(X~) when abits = 16);
  *   codes [T, C] uint8 (NULL = skip); h [T] fp32, z [T], argmax [T], argmin [T] int32
- *   (all NULL allowed when abits = 16). */
+ *   (all NULL allowed when abits = 16).  Rows of up to 32768 columns (OMQ_ERR_UNSUPPORTED beyond). */
 omq_status omq_act_quant_per_token(omq_stream_t stream, int64_t T, int64_t C, const float* X,
                                    const float* s, const float* delta, void* Xq, uint8_t* codes,
                                    float* h, int32_t* z, int32_t* argmax, int32_t* argmin,
@@ -129,7 +129,7 @@ omq_status omq_act_quant_per_token(omq_stream_t stream, int64_t T, int64_t C, co
 /* Straight-through backward of omq_act_quant_per_token, given dXq [T, C] fp32 and the saved
  * per-token state.  dX [T, C] fp32 = dL/dX; ds, ddelta [C] (NULL = skip) are the LET column sums
  * ds_i = -sum_t dX~_ti X~_ti / s_i and ddelta_i = -sum_t dX~_ti / s_i.  Needs a workspace of
- * omq_act_bwd_workspace_size bytes when ds or ddelta is requested. */
+ * omq_act_bwd_workspace_size bytes when ds or ddelta is requested.  Rows of up to 28672 columns. */
 omq_status omq_act_quant_per_token_bwd(omq_stream_t stream, int64_t T, int64_t C, const float* X,
                                        const float* s, const float* delta, const float* h,
                                        const int32_t* z, const int32_t* argmax,

@@ -352,7 +352,7 @@ __device__ __forceinline__ void act_row_state(const ActBwdArgs& a, int64_t t, fl
 template <int P, int NT, int VPT, int JB, int MINB, bool SUMS, bool RD = false>
 __global__ void __launch_bounds__(NT, MINB) act_bwd_stream(ActBwdArgs a) {
   constexpr bool LETP = (P == AP_LET || P == AP_RMS_LET);
-  static_assert(!(SUMS && P == AP_SWIGLU), "SwiGLU has no LET column sums");
+  static_assert(!SUMS || LETP, "only the LET producers have column sums");
   static_assert(VPT % JB == 0, "whole batches");
   constexpr int NE = SUMS ? 4 * VPT : 1;
   // the SwiGLU body is long: the batches of a long row, unrolled, overflow the instruction cache (2048 x 28672:
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(NT, MINB) act_bwd_stream(ActBwdArgs a) {
   // slots), computed once; the exact division of the quantizer input takes it too (omq_div2).  The RMSNorm
   // backward also keeps x * rstd and the masked gradient of its elements in registers for pass 2
   constexpr bool RS = SUMS;
-  constexpr bool KEEP = RS && P == AP_RMS_LET;
+  constexpr bool KEEP = RS && P == AP_RMS_LET && VPT <= 8;   // a longer row's would spill
   // the plain form with a.rowdot: D[head, t] = the sum of bf16(dX) X over each 128-column head (the
   // attention backward's rowsum(dO * O)), taken while the row is here; the float4 group j of a warp
   // is one head (lane L holds its columns 4L .. 4L + 3)
@@ -776,12 +776,13 @@ static omq_status act_bwd_go(cudaStream_t st, const ActBwdArgs& a0) {
   return OMQ_OK;
 }
 
-// Row length -> threads and vectors per thread.  Without LET column sums any length up to 28 K streams in
-// batches of four vectors; the column sums keep 8 VPT accumulators per thread in registers.
+// Row length -> threads and vectors per thread, up to 28 K columns.  Without LET column sums a row streams in
+// batches of four vectors; the column sums keep 8 VPT accumulators per thread in registers (past 16 K columns
+// 112 of them, of which 30 spill: 1531 x 28672 takes 334 us forward and backward, 1531 x 16384 160).
 template <int PRODUCER>
 static omq_status act_bwd_dispatch(cudaStream_t st, const ActBwdArgs& a) {
   const int64_t vpt = (a.C / 4 + 255) / 256;
-  const bool sums = PRODUCER != AP_SWIGLU && a.part_s != nullptr;
+  const bool sums = a.part_s != nullptr;
   if constexpr (PRODUCER == AP_PLAIN) {
     if (a.rowdot) {   // the row dot's partials take registers: loads in pairs to keep four CTAs per SM (two for longer rows)
       if (sums) return OMQ_ERR_UNSUPPORTED;
@@ -808,11 +809,12 @@ static omq_status act_bwd_dispatch(cudaStream_t st, const ActBwdArgs& a) {
     }
     return OMQ_ERR_UNSUPPORTED;
   }
-  if constexpr (PRODUCER != AP_SWIGLU) {
+  if constexpr (PRODUCER == AP_LET || PRODUCER == AP_RMS_LET) {
     if (vpt <= 4) return act_bwd_go<PRODUCER, 256, 4, 4, 2, true>(st, a);
     if (vpt <= 8) return act_bwd_go<PRODUCER, 512, 4, 4, 1, true>(st, a);
     if (vpt <= 12) return act_bwd_go<PRODUCER, 512, 6, 2, 1, true>(st, a);
     if (vpt <= 16) return act_bwd_go<PRODUCER, 512, 8, 2, 1, true>(st, a);
+    if (vpt <= 28) return act_bwd_go<PRODUCER, 512, 14, 2, 1, true>(st, a);
   }
   return OMQ_ERR_UNSUPPORTED;
 }

@@ -23,6 +23,10 @@ pytestmark = pytest.mark.gpu
     (33, 28672, 4, False),       # through shared memory, 1024 threads
     (9, 4104, 3, False),
     (5, 12288, 4, True),         # the row alone takes the 48 KB a CTA has without asking for more
+    (9, 16384, 4, True),
+    (11, 16392, 4, True),        # the longest form of the LET column sums
+    (310, 20488, 6, True),       # two rows a CTA and more
+    (7, 28672, 4, True),
     (640, 4096, 4, False),
 ])
 def test_act_row_edges(cuda_lib, T, C, nbits, let):
@@ -71,7 +75,17 @@ def test_swiglu_rows(cuda_lib, T, ffn):
 def test_long_rmsnorm_rows(cuda_lib, T, d):
     """RMSNorm rows of 512 and 1024 threads, of four and eight vectors each, in a block checked stage by stage."""
     shape = I.BlockShape(f"rms_{T}_{d}", T=T, d=d, n_heads=1, n_kv=1, ffn=128, wbits=4, abits=4, group=0,
-                         let=int(d <= 16384))          # LET column sums reach 16 K columns
+                         let=int(d <= 16384))
+    _, got = B._run(shape)
+    W, x, th, yfp = got["inputs"]
+    compare_step(shape, W, x, th, yfp, got["y"], got["loss"], {k: v for k, v in got.items() if k.startswith("d")},
+                 got["saved"], shape.name)
+
+
+@pytest.mark.parametrize("T,d", [(5, 16392), (3, 20480)])
+def test_longest_rmsnorm_rows_with_let(cuda_lib, T, d):
+    """RMSNorm rows past 16 K columns with LET: the column sums' longest form, whose second pass reads the row again."""
+    shape = I.BlockShape(f"rms_let_{T}_{d}", T=T, d=d, n_heads=1, n_kv=1, ffn=128, wbits=4, abits=4, group=0, let=1)
     _, got = B._run(shape)
     W, x, th, yfp = got["inputs"]
     compare_step(shape, W, x, th, yfp, got["y"], got["loss"], {k: v for k, v in got.items() if k.startswith("d")},
