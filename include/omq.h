@@ -178,6 +178,14 @@ omq_status omq_gemm_bf16(omq_stream_t stream, int64_t M, int64_t N, int64_t K, i
                          const float* bias, const float* R, int64_t ldr, float beta_acc,
                          int32_t causal, int32_t* dev_status);
 
+/* The output tile that a product of M x N over K takes on the current device: *columns by 128 rows on
+ * one CTA (*ctas = 1) or by 256 rows on a pair of CTAs (2).  lwc_group = 0: a plain product
+ * (omq_gemm_bf16 without batch or causal mode); > 0: a weight-gradient product with the LWC backward
+ * in its epilogue, M = Cout, N = Cin, K = tokens, groups of lwc_group columns (N = one per row);
+ * both outputs are 0 where the epilogue does not take such groups.  Pure host function, for tests and
+ * profiles.  OMQ_ERR_SHAPE for a non-positive size or a group that does not divide N. */
+omq_status omq_gemm_tile(int64_t M, int64_t N, int64_t K, int64_t lwc_group, int32_t* columns, int32_t* ctas);
+
 /* Failure-detection self-test (the paper has no counterpart): checks that a device-side wait
  * that never completes ends with OMQ_ERR_TIMEOUT instead of a hang.  Runs the tensor-core product
  * of omq_gemm_bf16, C [M, N] fp32 = A [M, K] B [N, K]^T (bf16, both K-major, rows packed; one

@@ -97,6 +97,7 @@ _SIGS = {
     "omq_block_loss_noalloc": (I32, [P, I64, P, P, P, P, P]),
     "omq_gemm_bf16": (I32, [P, I64, I64, I64, I64, P, I64, I64, I32, P, I64, I64, I32, P, P, I64, I64, F32,
                             P, P, I64, F32, I32, P]),
+    "omq_gemm_tile": (I32, [I64, I64, I64, I64, POINTER(c_int32), POINTER(c_int32)]),
     "omq_selftest_bounded_wait": (I32, [P, I64, I64, I64, P, P, P, ctypes.c_uint64, I32, P]),
     "omq_qlinear_fwd": (I32, [P, I64, I64, I64, P, P, P, P, P, P, P, P, P, P]),
     "omq_qlinear_bwd": (I32, [P, I64, I64, I64, P, P, P, P, P, P, P, P, P, P, P, P, P, P, SZ, P]),
@@ -268,6 +269,12 @@ def omq_attention_bwd(T, n_heads, n_kv, Q, ldq, K, V, ldkv, O, ldo, lse, dO, ldd
     check("omq_attention_bwd", lib().omq_attention_bwd(
         stream_handle(stream), T, n_heads, n_kv, ptr(Q), ldq, ptr(K), ptr(V), ldkv, ptr(O), ldo, ptr(lse), ptr(dO),
         lddo, ptr(D), ptr(dQ), ldg, ptr(dK), ptr(dV), ldgkv, ptr(dev_status)))
+
+
+def omq_gemm_tile(M, N, K, lwc_group=0):
+    columns, ctas = c_int32(), c_int32()
+    check("omq_gemm_tile", lib().omq_gemm_tile(M, N, K, lwc_group, ctypes.byref(columns), ctypes.byref(ctas)))
+    return columns.value, ctas.value
 
 
 def omq_qlinear_saved_sizes(T, Cin, Cout, cfg):

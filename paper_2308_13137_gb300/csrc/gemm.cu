@@ -1100,6 +1100,15 @@ extern "C" omq_status omq_gemm_bf16(omq_stream_t stream, int64_t M, int64_t N, i
   return gemm_launch((cudaStream_t)stream, M, N, K, batch, a, b, ep, causal, dev_status);
 }
 
+extern "C" omq_status omq_gemm_tile(int64_t M, int64_t N, int64_t K, int64_t lwc_group, int32_t* columns, int32_t* ctas) {
+  OMQ_REQUIRE(M > 0 && N > 0 && K > 0 && lwc_group >= 0 && (lwc_group == 0 || N % lwc_group == 0), OMQ_ERR_SHAPE);
+  OMQ_REQUIRE(columns && ctas, OMQ_ERR_INVALID_ARG);
+  const GemmTile t = lwc_group ? gemm_lwc_tile(M, N, K, lwc_group) : gemm_tile(M, N, K, 1, 0);
+  *columns = t.bn;
+  *ctas = t.bn == 0 ? 0 : t.pair ? 2 : 1;
+  return OMQ_OK;
+}
+
 // Failure-detection self-test: the product above on one CTA with every wait bounded by
 // wait_limit_ns, and optionally without its first operand load, so that the wait for it expires.
 extern "C" omq_status omq_selftest_bounded_wait(omq_stream_t stream, int64_t M, int64_t N, int64_t K, const void* A,

@@ -183,3 +183,12 @@ def test_qlinear_workspace_serves_every_configuration():
                  for g in (0, 8, 32, 64, 128, 256) for let in (0, 1)}
         sizes.add(L.omq_qlinear_workspace_size(T, Cin, Cout, None))
         assert len(sizes) == 1 and sizes.pop() > 2 * T * Cout + 4 * Cout * Cin + 4 * T * Cin
+
+
+def test_gemm_tile_query():
+    assert _lib.omq_gemm_tile(100, 8, 8) == (64, 1)
+    assert _lib.omq_gemm_tile(2048, 4096, 4096) == (256, 2)
+    assert _lib.omq_gemm_tile(512, 512, 256, 16) == (0, 0)        # the epilogue takes groups of 32 and more
+    for bad in ((0, 8, 8, 0), (8, 8, 0, 0), (8, 512, 8, 96), (8, 8, 8, -1)):
+        with pytest.raises(_lib.OmqError):
+            _lib.omq_gemm_tile(*bad)

@@ -20,7 +20,7 @@ pytestmark = pytest.mark.gpu
     (700, 5120, 4, True),        # 512 threads
     (40, 9000, 6, True),
     (30, 13000, 4, True),
-    (33, 28672, 4, False),       # through shared memory, 1024 threads
+    (33, 28672, 4, False),       # through shared memory, 512 threads
     (9, 4104, 3, False),
     (5, 12288, 4, True),         # the row alone takes the 48 KB a CTA has without asking for more
     (9, 16384, 4, True),

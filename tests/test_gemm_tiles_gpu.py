@@ -1,7 +1,7 @@
 """omq_gemm_bf16 at sizes that take each of its output tiles (single CTAs of 64, 128 and 256 columns, pairs
-of 128, 192 and 256), with ragged last tiles, and the weight-gradient product with the LWC epilogue
-at column counts that are no multiple of its 32-column chunk.  Operands are small integers, so
-every product and sum is exact in fp32 and the comparison is for equality."""
+of 128, 192 and 256), with ragged last tiles.  Operands are small integers, so every product and sum is
+exact in fp32 and the comparison is for equality.  The tile of each size is asserted, so that another cost model
+cannot leave one of them untested."""
 import pytest
 import torch
 
@@ -9,25 +9,28 @@ from paper_2308_13137_gb300 import _lib
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [   # M, N, K: the tile each is chosen for
-    (129, 136, 72),            # 64 columns
-    (412, 2048, 520),
-    (300, 4096, 200),          # 128 columns or pairs of 128
-    (512, 12288, 136),
-    (300, 12288, 264),         # 256 columns on one CTA
-    (1000, 6408, 328),
-    (1531, 4096, 776),         # pairs of 192
-    (2048, 4104, 1024),        # pairs of 256, ragged
-    (2048, 12288, 512),
-    (1531, 12288, 320),        # pairs of 256
-    (100, 8, 8),
-]
+TILES = {   # M, N, K: columns of the tile and its CTAs
+    (129, 136, 72): (64, 1),
+    (412, 2048, 520): (64, 1),
+    (100, 8, 8): (64, 1),
+    (300, 12288, 264): (128, 1),
+    (120, 22016, 136): (128, 1),
+    (120, 22016, 1032): (256, 1),
+    (300, 4096, 200): (128, 2),
+    (512, 12288, 136): (192, 2),
+    (1000, 6408, 328): (192, 2),
+    (1531, 4096, 776): (192, 2),
+    (2048, 4104, 1024): (256, 2),
+    (2048, 12288, 512): (256, 2),
+    (1531, 12288, 320): (256, 2),
+}
 
 
 @pytest.mark.parametrize("layout", [(1, 1), (1, 0), (0, 0)])
-@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("M,N,K", TILES)
 def test_gemm_tiles(cuda_lib, M, N, K, layout):
     ak, bk = layout
+    assert _lib.omq_gemm_tile(M, N, K) == TILES[M, N, K]
     if not ak and M % 8:
         M += 8 - M % 8
     g = torch.Generator(device="cuda").manual_seed(M + N + K)

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("T,Cin,Cout,abits,group,let", [
     (1, 64, 8, 16, 0, 0),            # one token, one column of tiles
     (129, 512, 264, 4, 0, 1),        # one row past a slab of the column sums
-    (300, 520, 136, 8, 0, 1),        # Cin not a multiple of 32: the separate pass
+    (300, 520, 136, 8, 0, 1),        # Cin not a multiple of the epilogue's 32-column chunk
     (260, 768, 512, 16, 128, 0),
     (127, 384, 200, 4, 64, 0),
     (200, 512, 256, 4, 128, 1),      # LET with groups: the separate pass
@@ -78,3 +78,23 @@ def test_flat_rows(cuda_lib, T, Cin, Cout, abits, group, let):
     """Every third row equal to 64 in the quantizer's input: its step is the floor, 1e-5, and its quotients, 6.4e6,
     are past the range of the fast rounding, next to rows that are inside."""
     test_qlinear_bwd_routes(cuda_lib, T, Cin, Cout, abits, group, let, flat=True)
+
+
+@pytest.mark.parametrize("T,Cin,Cout,group,let,tile", [
+    (130, 512, 120, 0, 1, (64, 1)),
+    (300, 768, 512, 32, 0, (64, 1)),
+    (1031, 1032, 1032, 0, 1, (128, 1)),      # ragged last tile and last chunk
+    (1031, 512, 3080, 0, 0, (128, 1)),
+    (260, 768, 512, 64, 0, (128, 1)),
+    (260, 768, 120, 128, 0, (256, 1)),
+    (260, 768, 512, 128, 0, (256, 2)),
+    (1531, 4104, 2048, 0, 1, (256, 2)),
+    (1531, 4096, 2048, 0, 0, (256, 2)),
+    (200, 512, 256, 128, 1, (0, 0)),         # LET with groups, groups of 16: the separate pass
+    (200, 512, 256, 16, 0, (0, 0)),
+])
+def test_lwc_epilogue_tiles(cuda_lib, T, Cin, Cout, group, let, tile):
+    """Every output tile of the weight-gradient product with the LWC epilogue, and the pass where it has none."""
+    if not (group and let):
+        assert _lib.omq_gemm_tile(Cout, Cin, T, group or Cin) == tile
+    test_qlinear_bwd_routes(cuda_lib, T, Cin, Cout, 4, group, let)
