@@ -311,8 +311,8 @@ __device__ __forceinline__ float2 omq_ste_dh2_small(float2 w, const QState& s, f
 struct MaxMin { float M; int iM; float m; int im; };
 
 constexpr int OMQ_NO_INDEX = 0x7fffffff;   // no element equals the extreme (yet)
-// The index a forward saves.  In a row or group of NaN alone no element equals the extreme: the index is then its
-// `first` column, because the backward reads and writes at it (a calibration that diverges returns NaN).
+// The index a forward saves.  In a row or group of NaN alone no element equals the extreme: the index is then one of
+// its columns, `first`, because the backward reads and writes at it (a calibration that diverges returns NaN).
 __device__ __forceinline__ int omq_saved_index(int i, int first) { return i == OMQ_NO_INDEX ? first : i; }
 
 __device__ __forceinline__ MaxMin mm_identity() { MaxMin r; r.M = -INFINITY; r.iM = OMQ_NO_INDEX; r.m = INFINITY; r.im = OMQ_NO_INDEX; return r; }

@@ -252,10 +252,12 @@ __global__ void __launch_bounds__(256, 4) lwc_fwd_kernel(LwcFwdArgs a) {
 // 8 (lwc_fwd_kernel<2>, which groups of 8 and 16 still take): the two sigmoids are formed by two lanes and
 // exchanged; without LET factors the extremes are taken on bf16 pairs and their first indices from equality
 // masks, one bit per column; the rounding stays off the conversion pipe (omq_rint2_small).  5120 x 5120
-// at 2 bits in groups of 64: 90 -> 24 us (about 18 at the HBM rate); the four weights of a 7B block in
-// groups of 128: 555 -> about 240 us, and 325 us less in that block's forward.
+// at 2 bits in groups of 64: 90 -> 26 us (17 at the HBM rate); the four weights of a 7B block in groups of 128:
+// 555 -> 217 us, and 325 us less in that block's forward.
+// Unscaled groups of 64 are held to 64 registers, four CTAs a SM: with 73, three CTAs, that weight's forward and
+// backward took 87.8 us instead of 84.3.
 template <int LPG, bool SCALED>
-__global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_t per_warp, int64_t total) {
+__global__ void __launch_bounds__(256, !SCALED && LPG == 2 ? 4 : 0) lwc_fwd_group_kernel(LwcFwdArgs a, int64_t per_warp, int64_t total) {
   constexpr int GPW = 32 / LPG, GSZ = 32 * LPG;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = lane & (LPG - 1), slot = lane / LPG;
@@ -328,8 +330,10 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
         if (sub & 1) ga = other;
       }
     }
-    // first column of the max and of the min: this lane's, then the group's
-    int iM = OMQ_NO_INDEX, im = OMQ_NO_INDEX;
+    // first column of the max and of the min: this lane's, then the group's.  A lane without one holds the group's
+    // last column, which is also what a group of NaN alone saves (omq_saved_index without a further step)
+    const int last = (int)col0 + GSZ - 1 - 8 * sub;
+    int iM = last, im = last;
     if constexpr (SCALED) {
 #pragma unroll
       for (int i = 31; i >= 0; --i) {
@@ -351,7 +355,7 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
         const uint32_t lo = mask & 0xffffu, hi = mask >> 16;
         const int i0 = lo ? 2 * (__ffs(lo) - 1) : 64, i1 = hi ? 2 * (__ffs(hi) - 1) + 1 : 64;
         const int i = min(i0, i1);
-        return i < 64 ? (int)col0 + (i >> 3) * LPG * 8 + (i & 7) : OMQ_NO_INDEX;
+        return i < 64 ? (int)col0 + (i >> 3) * LPG * 8 + (i & 7) : last;
       };
       iM = first(eM);
       im = first(em);
@@ -363,10 +367,7 @@ __global__ void __launch_bounds__(256) lwc_fwd_group_kernel(LwcFwdArgs a, int64_
     }
     const QState qs = omq_qstate(M, m, ga, gb, Q, a.eps);
     if (valid) {
-      if (sub == 0) {                            // col0 is the group's first column here
-        a.h[k] = qs.h; a.z[k] = (int32_t)qs.z;
-        a.imax[k] = omq_saved_index(iM, (int)col0); a.imin[k] = omq_saved_index(im, (int)col0);
-      }
+      if (sub == 0) { a.h[k] = qs.h; a.z[k] = (int32_t)qs.z; a.imax[k] = iM; a.imin[k] = im; }
       if (sub == LPG - 1) {
         if (a.ga_out) { a.ga_out[k] = ga; a.gb_out[k] = gb; }
         if (a.M_out) { a.M_out[k] = M; a.m_out[k] = m; }
@@ -839,8 +840,8 @@ __global__ void __launch_bounds__(LWC_BWD_THREADS, 3) lwc_bwd_tile_kernel(LwcBwd
 // Groups of 32 LPG columns without LET terms, laid out as in lwc_fwd_group_kernel: every lane holds 32 columns
 // of one group (weight and gradient in registers, all loads issued before the first use), the groups of the
 // matrix are one list, and the routing to the group's max / min is applied before dW~ is written.
-// 10 bytes per weight.  lwc_bwd_tile_kernel, one 8-column chunk a thread in flight, took 125 us for
-// 5120 x 5120 in groups of 64 (about 40 at the HBM rate).
+// 10 bytes per weight: 5120 x 5120 in groups of 64 takes 54 us (41 at the HBM rate); lwc_bwd_tile_kernel, one
+// 8-column chunk a thread in flight, took 125.
 template <int LPG>
 __global__ void __launch_bounds__(256) lwc_bwd_group_kernel(LwcBwdArgs a, int64_t total) {
   constexpr int GPW = 32 / LPG, GSZ = 32 * LPG;
