@@ -70,8 +70,8 @@ __device__ __forceinline__ void let_sub4(float (&v)[4], const ActFwdArgs& a, int
 // Rows of up to 4 K columns, one CTA a row, held in the registers of 128 threads (32 values each).  Two block
 // barriers (three with RMSNorm): the extremes are combined from per-warp values by every thread, and the first
 // indices are found by the holders of an extreme alone, in shared memory.  What bounds it is the latency of
-// its phases, so many short CTAs beat fewer with several rows each: 2048 x 4096 with LET takes 29 us, and 33,
-// 31, 33 and 40 with two, three, four and seven rows a CTA (17 against 19 - 23 without LET).  The rounding
+// its phases, so many short CTAs beat fewer with several rows each: 2048 x 4096 takes 25 us with LET and 13 without,
+// and with two, three, four and seven rows a CTA 14, 7, 14 and 38 % more (12 - 35 % without LET).  The rounding
 // stays off the conversion pipe.
 template <int P, int NT, int VPT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) act_fwd_rows(ActFwdArgs a) {
@@ -980,7 +980,7 @@ __global__ void __launch_bounds__(NT) qkv_fwd_rows(QkvArgs a) {
 // and sums the h path; the owner of each routed pair (the first max / min and its RoPE partner) then
 // rewrites that pair with the routing added.
 //
-// A CTA owns the pairs of all three segments (q | k | v, warps never straddle two), or of one segment where
+// A CTA owns the pairs of all three segments (q | k | v; with odd head counts a warp holds some of two), or of one where
 // three do not fit 512 threads x 4 pairs, and walks a slab of rows, the next one prefetched into L2.  The
 // quantizer states and the routed pairs of several rows are formed together, one warp each, so a row has no
 // chain of dependent loads and one barrier.  1/s_a of the thread's query columns is formed once a CTA: it
